@@ -582,6 +582,7 @@ constexpr int kRegWarps = kRegThreads / 32;
 constexpr int kRegMaxGroups = 8;
 constexpr int kGroupTokens = 4 * kRegThreads;
 constexpr int kBins = 2048;    // of a digit
+constexpr unsigned kZeroDigit = 0x80000000u >> 21;  // first digit of a score of 0
 constexpr int kHistReps = 4;   // histograms, each shared by 8 warps
 constexpr int kHistBytes = kHistReps * kBins * 4;
 constexpr int kMaxSelectCluster = 8;
@@ -890,7 +891,9 @@ __global__ void __maxnreg__(56) evict_select_smem_kernel(SelectArgs a, int JG) {
     unsigned remaining = (unsigned)k;
     // first digit: a token at or above the digit's upper bound joins the slice,
     // one below its lower bound the tail; the others stay in contention and
-    // count toward the second digit.  (A bound that is no number compares false.)
+    // count toward the second digit.  (A bound that is no number compares false.
+    // Comparisons flush subnormal operands to 0, and so were the scores: the
+    // digit of 0 ends at the smallest normal float, its own bound is subnormal.)
     choose_digit(whist, sh, remaining, C, 0);
     remaining = sh.remaining;
     bool done = sh.eqcount == remaining;  // every key with this digit is in the slice
@@ -899,7 +902,8 @@ __global__ void __maxnreg__(56) evict_select_smem_kernel(SelectArgs a, int JG) {
       const float flo = key_score(digit << 21);
       const float fhi = done ? flo
                              : digit == kBins - 1 ? __uint_as_float(0x7fffffffu)
-                                                  : key_score((digit + 1) << 21);
+                             : digit == kZeroDigit ? FLT_MIN
+                                                   : key_score((digit + 1) << 21);
 #pragma unroll 2
       for (int g = 0; g < JG; ++g) {
         const uint32_t l4 = (live >> (4 * g)) & 0xFu;

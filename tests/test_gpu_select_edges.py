@@ -39,6 +39,27 @@ def scores(kind, shape, seed):
         s[..., ::7] = 1e-42
         s[..., 5:405:8] = torch.finfo(torch.float32).max
         return s
+    if kind == "zeros":     # sparse scores: the k-th largest is 0
+        return torch.zeros(shape)
+    if kind == "few":       # 31 above 0, the others 0 of either sign
+        s = torch.zeros(shape)
+        s[..., 1::3] = -0.0
+        s[..., 50:3150:100] = torch.exp(torch.randn(s[..., 50:3150:100].shape, generator=g))
+        return s
+    if kind == "few_subnormal":
+        s = scores("few", shape, seed)
+        s[..., ::2][s[..., ::2] <= 0] = 1e-42
+        s[..., 1::4][s[..., 1::4] <= 0] = -1e-42
+        return s
+    if kind == "few_negative":  # 31 above 0, a quarter at 0, the others below
+        s = scores("few", shape, seed)
+        return torch.where((s > 0) | (torch.rand(shape, generator=g) < 0.25), s,
+                           -torch.rand(shape, generator=g))
+    if kind == "negative":  # the k-th largest below 0
+        s = -torch.rand(shape, generator=g)
+        s[..., 50:3150:100] = 0.5
+        s[..., 60:2060:100] = 0.0
+        return s
     return torch.exp(1.5 * torch.randn(shape, generator=g))
 
 
@@ -56,6 +77,17 @@ def scores(kind, shape, seed):
     (140000, 2000, 14000, "equal", False),     # ... of 5
     (170001, 3400, 17000, "lognormal", True),  # ... of 6
     (200001, 100, 20000, "close", False),      # ... of 7
+    (512, 10, 51, "zeros", False),
+    (4097, 80, 400, "zeros", True),
+    (8191, 500, 2000, "few", False),
+    (8192, 80, 2000, "few_subnormal", False),
+    (20000, 400, 2000, "few_negative", False),
+    (32768, 655, 3277, "few", True),
+    (32768, 100, 3277, "negative", False),
+    (65537, 1300, 6500, "zeros", False),       # ties of 0 across clusters
+    (100003, 5000, 25000, "few_negative", True),
+    (140000, 2000, 14000, "few_subnormal", False),
+    (200001, 100, 20000, "few", False),
 ])
 def test_select_at_digit_and_cluster_edges(E, N, k_head, budget, kind, systematic):
     B, H, cap = 1, 2, -(-(budget + 9 * int(budget ** 0.5) + 64) // 16) * 16
@@ -71,6 +103,7 @@ def test_select_at_digit_and_cluster_edges(E, N, k_head, budget, kind, systemati
     assert int(c.dev_status) == 0
     for h in range(H):
         u = s[0, h].numpy()
+        u = np.where(np.abs(u) < np.finfo(np.float32).tiny, np.float32(0), u)  # read as 0
         cert, _ = O.certainty_set(u, 4, 32, k_head)
         assert np.array_equal(mask[0, h].cpu().numpy().astype(bool), cert)
         ref, _, m = O.inclusion_probabilities(u, cert, budget, 1e-6)
@@ -89,3 +122,38 @@ def test_select_at_digit_and_cluster_edges(E, N, k_head, budget, kind, systemati
             kept = cert | (uni < ref.astype(np.float32))
             diff = np.flatnonzero(kept != np.isin(np.arange(N), idx))
             assert np.all(near[diff])
+
+
+def test_redraw_with_scores_of_zero(E):
+    """Re-eviction of ragged units from scores that are exactly 0 on most rows, as
+    variance contributions are on certain rows, fewer of them above 0 than the
+    top slice holds."""
+    B, H, d, cap, k_head, budget = 2, 2, 64, 4736, 819, 2048
+    g = torch.Generator().manual_seed(5)
+    n = torch.tensor([[4352, 4097], [1, 4736]], dtype=torch.int32)
+    s = torch.exp(torch.randn((B, H, cap), generator=g))
+    s[torch.rand((B, H, cap), generator=g) < 0.9] = 0.0
+    src, out = (E.alloc_compact(B, H, cap, d, torch.bfloat16, DEV) for _ in range(2))
+    src.K_c.copy_(torch.randn((B, H, cap, d), generator=g))
+    src.V_c.copy_(torch.randn((B, H, cap, d), generator=g))
+    src.logw_c.zero_()
+    src.idx_c.copy_(torch.arange(cap, dtype=torch.int32).mul(3).expand(B, H, cap))
+    src.n_kept.copy_(n)
+    des = E.design_for(batch=B, n_kv_heads=H, group=1, head_dim=d, n_ctx=cap, layer=3, seed=17,
+                       k_head=k_head, budget_tokens=budget)
+    E.ebd_reevict(des, s.to(DEV), src, out)
+    torch.cuda.synchronize()
+    assert int(out.dev_status) == 0
+    for b in range(B):
+        for h in range(H):
+            m = int(n[b, h])
+            ref = O.reevict_unit(
+                *(t[b, h, :m].double().cpu().numpy() for t in (src.K_c, src.V_c, src.logw_c)),
+                src.idx_c[b, h, :m].cpu().numpy(), s[b, h, :m].numpy(), n_sink=4, n_recent=32,
+                k_head=k_head, budget_tokens=budget, eps=1e-6, seed=17, layer=3, b=b, kvh=h,
+                capacity=cap)
+            near = ~ref.inner.certain & (np.abs(ref.inner.u - ref.inner.pi) < TIE_BAND)
+            got = out.idx_c[b, h, :int(out.n_kept[b, h])].cpu().numpy() // 3
+            assert np.all(np.diff(got) > 0)
+            diff = set(got.tolist()) ^ set(ref.inner.idx.tolist())
+            assert all(near[i] for i in diff)
