@@ -203,6 +203,7 @@ __global__ void __launch_bounds__(kFThreads) score_lse_f32_kernel(
   float* qs = fsm;
   float* ks = fsm + L::kQ;  // [2][kK]
   const int rank = csize > 1 ? (int)cluster_rank() : 0;
+  if (csize > 1) cluster_arrive_started();
   const int rt = blockIdx.x / csize, unit = rt / rtiles, r0 = (rt - unit * rtiles) * L::kRows;
   const int nk_all = (n_ctx + kFKeys - 1) / kFKeys;
   const int k0 = (int)((long long)rank * nk_all / csize);
@@ -270,6 +271,7 @@ __global__ void __launch_bounds__(kFThreads) score_lse_f32_kernel(
     lse_merge(M, S, part[1][r].x, part[1][r].y, sc);
   }
   if (csize > 1) {
+    cluster_wait_acquire();  // CTA 0 runs
     if (r < L::kRows) {
       const uint32_t dst = cluster_map(smem_u32(&lead[rank][r]), 0);
       asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(dst), "f"(M), "f"(S)
