@@ -369,14 +369,17 @@ static ebd_status launch_f32(Kernel kernel, long long grid, int cluster, int sme
   return cuda_status(cudaLaunchKernelEx(&cfg, kernel, args...));
 }
 
-// Clusters of `cluster` CTAs that this GPU holds at a time (a cluster lies
-// within one GPC, so that is fewer than SMs / cluster), asked once per device.
-template <typename Kernel>
-static int resident_clusters(Kernel kernel, int cluster, int smem, int slot) {
-  static std::atomic<int> cached[64][4];  // of this kernel, [device][log2 of the size]
+// Clusters of 2^lg CTAs of pass 1 that this GPU holds at a time (a cluster lies
+// within one GPC, so that is fewer than SMs / 2^lg; at d = 64 two CTAs share an
+// SM), asked once per device and kernel.
+template <int D, int I>
+static int resident_lse_clusters(int lg) {
+  static std::atomic<int> cached[64][4];
+  const auto kernel = score_lse_f32_kernel<D, I>;
+  const int cluster = 1 << lg, smem = F32Layout<D, I>::kLseBytes;
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return sm_count() / cluster;
-  int n = cached[dev][slot].load(std::memory_order_relaxed);
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return sm_count() >> lg;
+  int n = cached[dev][lg].load(std::memory_order_relaxed);
   if (n > 0) return n;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)cluster);
@@ -393,9 +396,9 @@ static int resident_clusters(Kernel kernel, int cluster, int smem, int slot) {
           cudaSuccess ||
       cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n < 1) {
     (void)cudaGetLastError();
-    n = sm_count() / cluster;
+    n = sm_count() >> lg;
   }
-  cached[dev][slot].store(n, std::memory_order_relaxed);
+  cached[dev][lg].store(n, std::memory_order_relaxed);
   return n;
 }
 
@@ -409,8 +412,7 @@ static double plan_lse_f32(int units, int n_ctx, int n_obs, double tile_us, int&
   for (int lg = 0; lg < 4; ++lg) {
     const int c = 1 << lg;
     if (lg > 0 && c > ktiles) break;
-    const long long fit =
-        resident_clusters(score_lse_f32_kernel<D, I>, c, F32Layout<D, I>::kLseBytes, lg);
+    const long long fit = resident_lse_clusters<D, I>(lg);
     const double cost = (double)((rts + fit - 1) / fit) * (3. + tile_us * ((ktiles + c - 1) / c));
     if (lg == 0 || cost < best) {
       best = cost;

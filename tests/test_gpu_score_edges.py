@@ -2,6 +2,10 @@
 (160-key tiles, 128-key items, chunks of at most 160 query rows, query rows
 resident up to 512 and streamed beyond, keys split over a cluster) and of the
 float32 kernels' tiles, against the float64 oracle."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -98,3 +102,29 @@ def test_scores_right_after_the_query_gather(E):
             Qs[i % 2][3, 3 * G:4 * G, Nq - P:].reshape(G * P, d).cpu().double().numpy(),
             K[3, 3].cpu().double().numpy())
         np.testing.assert_allclose(out[i][3, 3].cpu().double().numpy(), ref, rtol=E0_RTOL, atol=0)
+
+
+ORDER = """
+import hashlib, sys, torch
+from paper_2607_21475_gb300 import ebd as E
+def score(B, H, R, N, d):
+    g = torch.Generator().manual_seed(9)
+    K, q = torch.randn((B, H, N, d), generator=g), torch.randn((B, H, R, d), generator=g)
+    s = torch.empty((B, H, N), device="cuda")
+    E.ebd_score(q.cuda(), K.cuda(), s)
+    return s.cpu().numpy().tobytes()
+if sys.argv[1] == "after":
+    score(1, 1, 200, 3000, 64)
+print(hashlib.sha256(score(2, 4, 1600, 2048, 128)).hexdigest())
+"""
+
+
+def test_float32_scores_do_not_depend_on_what_was_scored_before(E):
+    """One d = 128 request (200 row tiles, more than fit at a time) in a fresh
+    process, and in one that scored a d = 64 request first, of whose CTAs two
+    share an SM: the same split, so the same bits."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    got = [subprocess.run([sys.executable, "-c", ORDER, how], cwd=root, capture_output=True,
+                          text=True, check=True, timeout=300).stdout.split()[-1]
+           for how in ("fresh", "after")]
+    assert got[0] == got[1]
