@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       mbar_arrive_expect_tx(q_full, L::kHalves * L::kQBox);
 #pragma unroll
       for (int h = 0; h < L::kHalves; ++h)
-        tma_load_2d(smem + h * L::kQBox, &tmQ, h * 64, unit * a.n_obs + mt * kTcRows1, q_full);
+        tma_load_3d(smem + h * L::kQBox, &tmQ, h * 64, mt * kTcRows1, unit, q_full);
       auto load_k = [&](int j) {
         const int s = j % KS;
         mbar_arrive_expect_tx(&k_full[s], L::kHalves * L::kKBox);
@@ -412,8 +412,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 #pragma unroll
           for (int h = 0; h < L::kHalves; ++h)
             for (int l = 0; l < nq_loads; ++l)
-              tma_load_2d(smem + h * L::kQBox + l * 256 * 128, &tmQ, h * 64,
-                          u * a.n_obs + l * 256, q_full);
+              tma_load_3d(smem + h * L::kQBox + l * 256 * 128, &tmQ, h * 64, l * 256, u, q_full);
           cur_u = u;
           qwait = true;
         }
@@ -715,9 +714,9 @@ __global__ void __launch_bounds__(kTsThreads, 1)
 #pragma unroll
           for (int h = 0; h < L::kHalves; ++h)
             for (int p = pa; p < pb; ++p)
-              tma_load_2d(smem + (stage * L::kHalves + h) * L::kQBox +
+              tma_load_3d(smem + (stage * L::kHalves + h) * L::kQBox +
                               (p - pa) * kTsQBoxRows * 128,
-                          &tmQ, h * 64, u * a.n_obs + p * kTsQBoxRows, &q_full[stage]);
+                          &tmQ, h * 64, p * kTsQBoxRows, u, &q_full[stage]);
         };
         for (int c = 0; c < nch; ++c, ++t) {
           const int qs = t % QS;
@@ -867,6 +866,23 @@ static PFN_cuTensorMapEncodeTiled_v12000 tc_encoder() {
   return fn;
 }
 
+// [units, rows, D] bf16, box = 64 columns x box_rows rows of one unit, 128-byte
+// swizzle.  Rows past a unit's last read as zeros: an accumulator column of
+// the padding adds 2^(0 - infinity) = 0, whatever the next unit's rows hold (a
+// NaN there would reach this unit's sums).
+static bool encode_bf16_units(CUtensorMap* map, const void* base, int units, int rows, int D,
+                              int box_rows) {
+  auto enc = tc_encoder();
+  if (!enc) return false;
+  const cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)rows, (cuuint64_t)units};
+  const cuuint64_t strides[2] = {(cuuint64_t)D * 2, (cuuint64_t)rows * D * 2};
+  const cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box,
+             estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // [rows, D] bf16 as 2D; box = 64 columns x box_rows rows, 128-byte swizzle.
 static bool encode_bf16_rows(CUtensorMap* map, const void* base, long long rows, int D,
                              int box_rows) {
@@ -921,10 +937,10 @@ static ebd_status launch_score_tc_t(int units, int n_ctx, int n_obs, const void*
                                     int32_t* dev_status, cudaStream_t s) {
   const bool stream = n_obs > kTcMaxRows;
   CUtensorMap tmQ1, tmK1, tmQ2, tmK2;
-  const long long qrows = (long long)units * n_obs, krows = (long long)units * n_ctx;
-  if (!encode_bf16_rows(&tmQ1, q_obs, qrows, D, kTcRows1) ||
+  const long long krows = (long long)units * n_ctx;
+  if (!encode_bf16_units(&tmQ1, q_obs, units, n_obs, D, kTcRows1) ||
       !encode_bf16_rows(&tmK1, K, krows, D, kTcKeys1) ||
-      !encode_bf16_rows(&tmQ2, q_obs, qrows, D, stream ? kTsQBoxRows : 256) ||
+      !encode_bf16_units(&tmQ2, q_obs, units, n_obs, D, stream ? kTsQBoxRows : 256) ||
       !encode_bf16_rows(&tmK2, K, krows, D, kTcKeys2))
     return EBD_ERR_CUDA;
   TcArgs a;

@@ -128,3 +128,25 @@ def test_float32_scores_do_not_depend_on_what_was_scored_before(E):
                           text=True, check=True, timeout=300).stdout.split()[-1]
            for how in ("fresh", "after")]
     assert got[0] == got[1]
+
+
+@pytest.mark.parametrize("R,N,d,dtype", [
+    (513, 300, 128, torch.bfloat16),   # streamed rows, 63 of padding in the last block
+    (1000, 129, 64, torch.bfloat16),
+    (450, 300, 128, torch.bfloat16),   # resident rows, two accumulators
+    (33, 700, 64, torch.bfloat16),
+    (70, 300, 128, torch.float32),
+])
+def test_a_unit_with_nan_leaves_its_neighbours_alone(E, R, N, d, dtype):
+    """The middle one of three units holds NaN in every query row and key: the
+    other two get the scores they get without it."""
+    g = torch.Generator().manual_seed(R)
+    K = torch.randn((1, 3, N, d), generator=g).to(dtype).to(DEV)
+    q = torch.randn((1, 3, R, d), generator=g).to(dtype).to(DEV)
+    ref, got = torch.empty((1, 3, N), device=DEV), torch.empty((1, 3, N), device=DEV)
+    E.ebd_score(q, K, ref)
+    q[0, 1] = float("nan")
+    K[0, 1] = float("nan")
+    E.ebd_score(q, K, got)
+    assert torch.isfinite(ref).all()
+    assert torch.equal(got[:, ::2], ref[:, ::2])
