@@ -136,11 +136,11 @@ constexpr int kCtmStages = 3;
 
 template <int D, bool SPARE>
 __global__ void __launch_bounds__(kCtmWarps * 32)
-    contrib_mma_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16* __restrict__ Kc,
-                       const __nv_bfloat16* __restrict__ Vc, const float* __restrict__ logw,
-                       const int32_t* __restrict__ n_kept, const float* __restrict__ y,
-                       const float* __restrict__ lse, int group, int cap, int ctas,
-                       float* __restrict__ contrib) {
+    contrib_mma_kernel(const __nv_bfloat16* Q, const __nv_bfloat16* Kc,
+                       const __nv_bfloat16* Vc, const float* logw,
+                       const int32_t* n_kept, const float* y,
+                       const float* lse, int group, int cap, int ctas,
+                       float* contrib) {
   constexpr int kBox = 16 * 128;                 // 16 rows x 128 B (64 columns)
   constexpr int kHalves = D / 64;
   constexpr int kTile = 2 * kHalves * kBox;      // K then V
@@ -346,9 +346,9 @@ __global__ void __launch_bounds__(kCtmWarps * 32)
 constexpr int kBlkThreads = 128, kBlkRows = 4096;
 
 __global__ void __launch_bounds__(kBlkThreads)
-    block_scores_kernel(const float* __restrict__ contrib, const int32_t* __restrict__ idx_c,
-                        const int32_t* __restrict__ n_kept, int group, int cap, int block,
-                        int n_blocks, float* __restrict__ out) {
+    block_scores_kernel(const float* contrib, const int32_t* idx_c,
+                        const int32_t* n_kept, int group, int cap, int block,
+                        int n_blocks, float* out) {
   __shared__ int start[kBlkThreads + 1], range[2];
   __shared__ float buf[kBlkRows];
   grid_dependency_wait();

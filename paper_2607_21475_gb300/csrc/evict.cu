@@ -789,7 +789,7 @@ __global__ void __maxnreg__(56) evict_select_smem_kernel(SelectArgs a, int JG) {
   const int b = unit / a.n_kv_heads;
   const int kvh = unit - b * a.n_kv_heads;
   const int Nrow = a.n_ctx;
-  const int N = a.n_len ? min(max(__ldg(a.n_len + unit), 0), Nrow) : Nrow;
+  const int N = a.n_len ? min(max(a.n_len[unit], 0), Nrow) : Nrow;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const float* sp = a.scores + (size_t)unit * Nrow;
   const int ns = min(a.n_sink, N);
@@ -833,12 +833,12 @@ __global__ void __maxnreg__(56) evict_select_smem_kernel(SelectArgs a, int JG) {
     if (g < JG) {
       const int i0 = tok(g, 0);
       if (a.vec4 && i0 + 3 < N) {
-        raw[g] = __ldg(reinterpret_cast<const float4*>(sp + i0));
+        raw[g] = *reinterpret_cast<const float4*>(sp + i0);
       } else {
-        if (i0 < N) raw[g].x = __ldg(sp + i0);
-        if (i0 + 1 < N) raw[g].y = __ldg(sp + i0 + 1);
-        if (i0 + 2 < N) raw[g].z = __ldg(sp + i0 + 2);
-        if (i0 + 3 < N) raw[g].w = __ldg(sp + i0 + 3);
+        if (i0 < N) raw[g].x = sp[i0];
+        if (i0 + 1 < N) raw[g].y = sp[i0 + 1];
+        if (i0 + 2 < N) raw[g].z = sp[i0 + 2];
+        if (i0 + 3 < N) raw[g].w = sp[i0 + 3];
       }
     }
   }
@@ -1272,8 +1272,8 @@ constexpr int kGatherThreads = 128;  // small CTAs also fit beside a select CTA
 constexpr int kGatherUnroll = 4;
 
 __global__ void __launch_bounds__(kGatherThreads) gather_rows_kernel(
-    const uint4* __restrict__ K, const uint4* __restrict__ V, uint4* __restrict__ Kc,
-    uint4* __restrict__ Vc, const int32_t* __restrict__ idx_c, const int32_t* __restrict__ n_kept,
+    const uint4* K, const uint4* V, uint4* Kc,
+    uint4* Vc, const int32_t* idx_c, const int32_t* n_kept,
     int n_ctx, int cap, int cpr, int unit0) {
   // a programmatic dependent of the select that writes idx and n_kept
   grid_dependency_wait();
@@ -1304,8 +1304,8 @@ __global__ void __launch_bounds__(kGatherThreads) gather_rows_kernel(
         ok[u] = (unsigned)r < (unsigned)n_ctx;
         const size_t src = src_base + (size_t)(ok[u] ? r : 0) * cpr + ch;
         dst[u] = dst_base + (size_t)p * cpr + ch;
-        kv[u] = __ldg(K + src);
-        vv[u] = __ldg(V + src);
+        kv[u] = K[src];
+        vv[u] = V[src];
       }
     }
 #pragma unroll

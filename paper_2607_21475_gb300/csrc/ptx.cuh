@@ -116,6 +116,9 @@ __device__ __forceinline__ int ld_cg_s32(const int32_t* p) {
 // serialization may start while its predecessor in the stream runs; it must
 // wait before reading the predecessor's outputs or writing anything.  A
 // kernel lets its own dependents launch early with launch_dependents.
+// What the predecessor may write is read with plain loads: the read-only path
+// (__ldg, const __restrict__) is for data that does not change while the kernel
+// is resident, and such a load may move above the wait.
 __device__ __forceinline__ void grid_launch_dependents() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }

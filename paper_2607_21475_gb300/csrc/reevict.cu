@@ -19,11 +19,11 @@ constexpr int kComposeThreads = 256;
 // One warp per unit: row n_kept of K_c/V_c <- the new key/value (16-byte
 // chunks), log(1/pi) = 0, token position; n_kept + 1.
 __global__ void __launch_bounds__(kAppendWarps * 32)
-    append_kernel(const uint4* __restrict__ k_new, const uint4* __restrict__ v_new,
-                  const int32_t* __restrict__ positions, int units, int n_kv_heads, int cpr,
-                  int cap, uint4* __restrict__ K_c, uint4* __restrict__ V_c,
-                  float* __restrict__ logw_c, int32_t* __restrict__ idx_c,
-                  int32_t* __restrict__ n_kept, int32_t* dev_status) {
+    append_kernel(const uint4* k_new, const uint4* v_new,
+                  const int32_t* positions, int units, int n_kv_heads, int cpr,
+                  int cap, uint4* K_c, uint4* V_c,
+                  float* logw_c, int32_t* idx_c,
+                  int32_t* n_kept, int32_t* dev_status) {
   // a decode launched next as a programmatic dependent may start its launch
   // now; it waits for this kernel's writes before reading the cache.  This
   // kernel is one itself, of whatever wrote the cache
@@ -33,6 +33,7 @@ __global__ void __launch_bounds__(kAppendWarps * 32)
   const int lane = threadIdx.x & 31;
   if (unit >= units) return;
   const int n = max(n_kept[unit], 0);
+  const int32_t pos = positions[unit / n_kv_heads];
   __syncwarp();
   if (n < cap) {
     const size_t dst = ((size_t)unit * cap + n) * cpr;
@@ -42,7 +43,7 @@ __global__ void __launch_bounds__(kAppendWarps * 32)
     }
     if (lane == 0) {
       logw_c[(size_t)unit * cap + n] = 0.f;
-      idx_c[(size_t)unit * cap + n] = positions[unit / n_kv_heads];
+      idx_c[(size_t)unit * cap + n] = pos;
     }
   } else if (lane == 0) {
     raise_status(dev_status, EBD_DEV_CAPACITY);
@@ -56,9 +57,9 @@ __global__ void __launch_bounds__(kAppendWarps * 32)
 // its scattered reads hold the row copies up, 108 -> 122 us for a redraw step of
 // 64 units x 4352 rows.)
 __global__ void __launch_bounds__(kComposeThreads)
-    compose_kernel(const float* __restrict__ logw_in, const int32_t* __restrict__ idx_in,
-                   int cap_in, const int32_t* __restrict__ n_kept_out, int cap_out,
-                   float* __restrict__ logw_out, int32_t* __restrict__ idx_out) {
+    compose_kernel(const float* logw_in, const int32_t* idx_in,
+                   int cap_in, const int32_t* n_kept_out, int cap_out,
+                   float* logw_out, int32_t* idx_out) {
   grid_dependency_wait();
   grid_launch_dependents();
   const int unit = blockIdx.y;
@@ -68,8 +69,10 @@ __global__ void __launch_bounds__(kComposeThreads)
     const size_t o = (size_t)unit * cap_out + p;
     const int j = idx_out[o];  // resident position in the input cache, < cap_in
     const size_t i = (size_t)unit * cap_in + j;
-    logw_out[o] += logw_in[i];
-    idx_out[o] = idx_in[i];
+    const float lw = logw_out[o] + logw_in[i];  // every load before the first store
+    const int32_t t = idx_in[i];
+    logw_out[o] = lw;
+    idx_out[o] = t;
   }
 }
 

@@ -194,8 +194,8 @@ __device__ __forceinline__ void lse_merge(float& M, float& S, float M2, float S2
 
 template <int D, int I>
 __global__ void __launch_bounds__(kFThreads) score_lse_f32_kernel(
-    const float* __restrict__ q_obs, const float* __restrict__ K, int n_ctx, int n_obs, int rtiles,
-    int csize, float sc, float* __restrict__ lse2) {
+    const float* q_obs, const float* K, int n_ctx, int n_obs, int rtiles,
+    int csize, float sc, float* lse2) {
   using L = F32Layout<D, I>;
   extern __shared__ __align__(16) float fsm[];
   __shared__ float2 part[2][L::kRows];  // the two warp columns' parts of a row
@@ -290,8 +290,8 @@ __global__ void __launch_bounds__(kFThreads) score_lse_f32_kernel(
 
 template <int D, int I>
 __global__ void __launch_bounds__(kFThreads) score_col_f32_kernel(
-    const float* __restrict__ q_obs, const float* __restrict__ K, int n_ctx, int n_obs, int ktiles,
-    float sc, const float* __restrict__ lse2, float* __restrict__ scores) {
+    const float* q_obs, const float* K, int n_ctx, int n_obs, int ktiles,
+    float sc, const float* lse2, float* scores) {
   using L = F32Layout<D, I>;
   extern __shared__ __align__(16) float fsm[];
   __shared__ float part[2][kFKeys];  // the two warp rows' parts of a key's sum
