@@ -1372,6 +1372,10 @@ int select_cluster_size(int n_ctx, int units) {
   return C;
 }
 
+// The most dynamic shared memory of the two select kernels (allow_smem).
+constexpr int kSelectSmem = kRegMaxGroups * kRegThreads * (int)sizeof(float4) + kHistBytes;
+constexpr int kBigSelectSmem = kMaxCtx / 8 + kSelWarps * 256 * 4;
+
 ebd_status launch_select_range(const ebd_design* d, const float* scores, const int32_t* n_len,
                                float* pi, uint8_t* mask, int32_t* idx_c, float* logw_c,
                                int32_t* n_kept, int cap, int32_t* dev_status, int unit0,
@@ -1408,9 +1412,7 @@ ebd_status launch_select_range(const ebd_design* d, const float* scores, const i
     const int per = (d->n_ctx + C - 1) / C;
     const int jg = (per + kGroupTokens - 1) / kGroupTokens;
     const size_t smem = (size_t)jg * kRegThreads * sizeof(float4) + kHistBytes;
-    if (cudaFuncSetAttribute(evict_select_smem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem) != cudaSuccess)
-      return EBD_ERR_CUDA;
+    if (allow_smem(evict_select_smem_kernel, kSelectSmem) != EBD_OK) return EBD_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(units * C));
     cfg.blockDim = dim3(kRegThreads);
@@ -1434,9 +1436,7 @@ ebd_status launch_select_range(const ebd_design* d, const float* scores, const i
     // the limit is set on every launch: with the kernel's static shared memory
     // even 48 KB of dynamic memory is above the default
     const size_t smem = (size_t)groups * kRegThreads * sizeof(float4) + kHistBytes;
-    if (cudaFuncSetAttribute(evict_select_smem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem) != cudaSuccess)
-      return EBD_ERR_CUDA;
+    if (allow_smem(evict_select_smem_kernel, kSelectSmem) != EBD_OK) return EBD_ERR_CUDA;
     if (dependent)
       return launch_dependent(evict_select_smem_kernel, dim3((unsigned)units), kRegThreads, smem,
                               stream, a, groups);
@@ -1446,9 +1446,7 @@ ebd_status launch_select_range(const ebd_design* d, const float* scores, const i
   // certainty bits (padded to 16 bytes), then the per-warp first-digit histograms
   const int words_pad = ((d->n_ctx + 31) / 32 + 3) & ~3;
   const size_t smem = (size_t)words_pad * 4 + (size_t)kSelWarps * 256 * 4;
-  if (cudaFuncSetAttribute(evict_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem) != cudaSuccess)
-    return EBD_ERR_CUDA;
+  if (allow_smem(evict_select_kernel, kBigSelectSmem) != EBD_OK) return EBD_ERR_CUDA;
   evict_select_kernel<<<units, kSelThreads, smem, stream>>>(a, words_pad);
   return launch_status();
 }

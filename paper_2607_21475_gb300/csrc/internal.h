@@ -14,6 +14,15 @@ inline ebd_status cuda_status(cudaError_t e) { return e == cudaSuccess ? EBD_OK 
 // Last launch error of this thread, mapped to a status (clears the error).
 inline ebd_status launch_status() { return cuda_status(cudaGetLastError()); }
 
+// Dynamic shared memory that launches of `kernel` may ask for.  The limit is the
+// process's, not the launch's: every call for a kernel passes the same number, its
+// largest layout, so that no thread lowers it between another's call and launch.
+template <typename Kernel>
+ebd_status allow_smem(Kernel kernel, int most) {
+  return cuda_status(
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+}
+
 // Launch as a programmatic dependent of what precedes it in the stream (the
 // kernel waits for that before it reads or writes memory).
 template <typename... Params, typename... Args>
