@@ -81,6 +81,10 @@ CASES = [
      (22.30e-7, 5.28e-7, 14.76e-7, 4.63e-7)),
     (32, 8, 4, 128, 1000, 1344, False, BF, 3.0, 2,
      (16.20e-7, 8.85e-7, 23.27e-7, 7.60e-7)),
+    (4, 8, 2, 64, 9000, 9501, False, BF, 1.0, 6,
+     (3.08e-7, 3.18e-7, 3.05e-7, 2.81e-7)),
+    (4, 8, 8, 128, 1500, 1801, False, BF, 3.0, 6,
+     (4.09e-7, 4.12e-7, 13.11e-7, 3.80e-7)),
 ]
 
 
