@@ -84,3 +84,25 @@ def test_exact_range_term_when_one_row_dominates(E, G, d, cap, mean, scale):  # 
             # (||y_hat|| of a dominated head), times p <= 1
             tol = 1e-5 * dec.b_exact + 2.0 ** -16 * np.linalg.norm(dec.y, axis=1)
             assert np.all(np.abs(got - dec.b_exact) <= tol)
+
+
+@pytest.mark.parametrize("G,d,cap", [(4, 128, 1600), (7, 128, 1601), (8, 64, 304)])
+def test_exact_range_term_of_small_tail_weights(E, G, d, cap):  # noqa: F811
+    """A certain row that takes all but 1e-25 of the weight: the tail's range term
+    is as small, and has its float32 digits all the same (the logits, 60 apart,
+    round by up to 4e-6 each)."""
+    B, H = 1, 2
+    Kc, Vc, logw, n = _synthetic_cache(B, H, cap, d, torch.bfloat16, "random", 5)
+    g = torch.Generator().manual_seed(6)
+    Q = torch.randn((B, H * G, d), generator=g).to(torch.bfloat16)
+    Q[..., 0], Kc[..., 0] = 16.0, 0.0
+    Kc[:, :, 50, 0] = 60.0 * d ** 0.5 / 16.0
+    logw[:, :, 50] = 0.0
+    out = _decode(E, Q.to(DEV), Kc.to(DEV), Vc.to(DEV), logw.to(DEV), n.to(DEV), True)
+    for h in range(H):
+        k = int(n[0, h])
+        dec = O.hajek_decode(Q[0, h * G:(h + 1) * G].double().numpy(),
+                             Kc[0, h, :k].double().numpy(), Vc[0, h, :k].double().numpy(),
+                             logw[0, h, :k].double().numpy())
+        assert np.all(dec.b_exact > 0) and np.all(dec.b_exact < 1e-20)
+        np.testing.assert_allclose(out[3][0, h * G:(h + 1) * G], dec.b_exact, rtol=2e-5)
