@@ -106,3 +106,36 @@ def test_exact_range_term_of_small_tail_weights(E, G, d, cap):  # noqa: F811
                              logw[0, h, :k].double().numpy())
         assert np.all(dec.b_exact > 0) and np.all(dec.b_exact < 1e-20)
         np.testing.assert_allclose(out[3][0, h * G:(h + 1) * G], dec.b_exact, rtol=2e-5)
+
+
+def test_exact_range_term_takes_no_longer_when_values_share_a_mean(E):  # noqa: F811
+    """Values with a mean of 256 times their spread on every channel: the rows that
+    the range pass has to evaluate one by one stay few, so the call takes about the
+    time it takes without the mean (every one of them: several times that)."""
+    B, H, G, d, cap = 4, 8, 5, 128, 2960
+    g = torch.Generator().manual_seed(7)
+    K, V = (torch.randn((B, H, cap, d), generator=g).to(torch.bfloat16).to(DEV) for _ in range(2))
+    Q = torch.randn((B, H * G, d), generator=g).to(torch.bfloat16).to(DEV)
+    lw = torch.rand((B, H, cap), generator=g).add(0.1).to(DEV)
+    n = torch.full((B, H), 2460, dtype=torch.int32, device=DEV)
+    y = torch.empty((B, H * G, d), device=DEV)
+    o = [torch.empty((B, H * G), device=DEV) for _ in range(4)]
+    ws = torch.empty(E.ebd_decode_workspace_bytes(E.EBD_BF16, B, H, G, d, cap), dtype=torch.uint8,
+                     device=DEV)
+
+    def microseconds(mean):
+        Vm = (V.float() + mean).to(torch.bfloat16)
+        best = float("inf")
+        for _ in range(5):
+            t0, t1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            for k in range(60):
+                if k == 10:
+                    t0.record()
+                E.ebd_certified_decode(Q, K, Vm, lw, n, y, *o, range_mode=E.EBD_RANGE_EXACT,
+                                       workspace=ws)
+            t1.record()
+            torch.cuda.synchronize()
+            best = min(best, t0.elapsed_time(t1) * 20)
+        return best
+
+    assert microseconds(256.0) <= 1.5 * microseconds(0.0)
