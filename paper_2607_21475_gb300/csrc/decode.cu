@@ -270,10 +270,10 @@ __global__ void __launch_bounds__(kReduceWarps * 32) decode_reduce_kernel(Reduce
 #pragma unroll
     for (int e = 0; e < PER; ++e) a.y[(size_t)hq * D + PER * lane + e] = 0.f;
     if (lane == 0) {
-      a.lse[hq] = -INFINITY;
       a.var[hq] = 0.f;
       a.b_t[hq] = 0.f;
       a.radius[hq] = 0.f;
+      HeadNorm{a.lse, a.radius, a.exact}.write(hq, -INFINITY, 0.f);
     }
     return;
   }
@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(kReduceWarps * 32) decode_reduce_kernel(Reduce
 #pragma unroll
   for (int e = 0; e < PER; ++e) a.y[(size_t)hq * D + PER * lane + e] = yv[e];
   if (lane == 0) {
-    a.lse[hq] = Mx + logf(l);
+    HeadNorm{a.lse, a.radius, a.exact}.write(hq, Mx, l);
     a.var[hq] = var;
     if (a.exact) {
       a.b_t[hq] = 0.f;  // filled by the exact range pass
@@ -331,7 +331,7 @@ __global__ void __launch_bounds__(kGenThreads) decode_exact_range_kernel(DecodeA
   const T* Kc = (const T*)a.Kc + (size_t)unit * a.cap * D;
   const T* Vc = (const T*)a.Vc + (size_t)unit * a.cap * D;
   const float* lw = a.logw + (size_t)unit * a.cap;
-  float q[GM][E], yv[GM][E], lse[GM], best[GM];
+  float q[GM][E], yv[GM][E], M[GM], l[GM], best[GM];
 #pragma unroll
   for (int g = 0; g < GM; ++g) {
 #pragma unroll
@@ -339,7 +339,8 @@ __global__ void __launch_bounds__(kGenThreads) decode_exact_range_kernel(DecodeA
       q[g][j] = g < G ? to_f32(Q[(size_t)g * D + lane + 32 * j]) * scale : 0.f;
       yv[g][j] = g < G ? a.y[(hq0 + g) * D + lane + 32 * j] : 0.f;
     }
-    lse[g] = g < G ? a.lse[hq0 + g] : 0.f;
+    M[g] = g < G ? a.radius[hq0 + g] : 0.f;
+    l[g] = g < G ? a.lse[hq0 + g] : 1.f;
     best[g] = 0.f;
   }
   for (int t = t0 + warp; t < t1; t += kGenWarps) {
@@ -362,9 +363,8 @@ __global__ void __launch_bounds__(kGenThreads) decode_exact_range_kernel(DecodeA
         const float dv = v[j] - yv[g][j];
         dist = fmaf(dv, dv, dist);
       }
-      const float x = warp_sum(dot) + lwt;
       dist = warp_sum(dist);
-      const float p = expf(x - lse[g]);  // w_i / N_hat
+      const float p = expf((warp_sum(dot) - M[g]) + lwt) / l[g];  // w_i / N_hat
       best[g] = fmaxf(best[g], sq * p * sqrtf(dist));
     }
   }
@@ -396,6 +396,7 @@ __global__ void decode_radius_kernel(ReduceArgs a, int n_heads) {
   yy = warp_sum(yy);
   if (lane == 0) {
     const float bt = a.b_t[hq], var = a.var[hq];
+    a.lse[hq] = a.radius[hq] + logf(a.lse[hq]);  // M + log l (HeadNorm)
     a.radius[hq] = (sqrtf(2.f * var * a.log_inv_delta) + bt * a.log_inv_delta) / (sqrtf(yy) + a.eps0);
   }
 }
@@ -572,7 +573,7 @@ extern "C" ebd_status ebd_certified_decode(ebd_dtype dtype, int32_t batch, int32
     a.lse = r.lse = lse + h0;
     r.var = var_hat + h0;
     a.b_t = r.b_t = b_t + h0;
-    r.radius = radius + h0;
+    a.radius = r.radius = radius + h0;
     const int n_heads = (int)(units * a.group);
     ebd_status st = EBD_ERR_UNSUPPORTED;
     const bool fast = plan.fast && fast_decode_usable(a, r, (int)units);
@@ -602,7 +603,8 @@ extern "C" ebd_status ebd_certified_decode(ebd_dtype dtype, int32_t batch, int32
     }
   }
   if (!r.exact) return EBD_OK;
-  // the radius of every query head from its V_hat and exact range term
+  // log N_hat and the radius of every query head, the latter from its V_hat and
+  // exact range term
   r.group = r.gstride = group;
   r.y = y;
   r.lse = lse;

@@ -60,6 +60,20 @@ __device__ __forceinline__ void finish_head(const float (&o)[PER], const float (
   var = fmaxf(0.f, (A2 - 2.f * yca + ycyc * U) / (l * l));
 }
 
+// log N_hat = M + log l of a head.  EBD_RANGE_EXACT: the range pass weighs its rows
+// by exp(logit - M) / l, since a log N_hat rounded to 32 bits puts up to half a unit
+// of its own size, 5e-7 at 8 to 16, on every weight.  M and l wait for it in the
+// head's radius and lse, which decode_radius_kernel then finishes.
+struct HeadNorm {
+  float* lse;
+  float* radius;
+  bool exact;
+  __device__ __forceinline__ void write(long long hq, float M, float l) const {
+    lse[hq] = exact ? l : M + logf(l);
+    if (exact) radius[hq] = M;
+  }
+};
+
 // One partial record per (unit, split slot, query head of the group), floats:
 //   [M, l, U, A2, cmax, umax, pad, pad, o[0..D), A1[0..D)]
 // (16-byte multiple, so o and A1 can be read as float4).  w-terms (l, o,
@@ -91,7 +105,8 @@ struct DecodeArgs {
   int tokens_per_split;   // CUDA-core path: token range of one split
   float* part;            // [units, splits, G, rec_floats(D)]
   float* y;               // exact range pass: final y_hat (read)
-  float* lse;             // exact range pass: final lse (read)
+  float* lse;             // exact range pass: l (read; HeadNorm)
+  float* radius;          // exact range pass: M (read; HeadNorm)
   float* b_t;             // exact range pass: running max (atomicMax)
   int32_t* dev_status;
 };

@@ -289,7 +289,8 @@ struct SecondArgs {
   const float* logw;
   const int32_t* n_kept;
   const float* y;
-  const float* lse;
+  const float* lse;  // RANGE: l
+  const float* m;    // RANGE: M (HeadNorm)
   float* out;  // contributions [units * gstride, cap], or b_t [units * gstride] (maximum)
   int cap;
   int group;
@@ -331,10 +332,12 @@ __global__ void __launch_bounds__(kCoreThreads) second_pass_kernel(SecondArgs a)
     qs[i / D][i % D] = in ? to_f32(Q[i]) * scale : 0.f;
     ys[i / D][i % D] = in ? a.y[hq0 * D + i] : 0.f;
   }
-  float ls[HP], best[HP];
+  float ls[HP], ln[HP], best[HP];  // log N_hat, or (RANGE) M and l
 #pragma unroll
   for (int h = 0; h < HP; ++h) {
-    ls[h] = warp + 4 * h < G ? a.lse[hq0 + warp + 4 * h] : 0.f;
+    const bool in = warp + 4 * h < G;
+    ls[h] = in ? (RANGE ? a.m : a.lse)[hq0 + warp + 4 * h] : 0.f;
+    ln[h] = RANGE && in ? a.lse[hq0 + warp + 4 * h] : 1.f;
     best[h] = 0.f;
   }
   if constexpr (!RANGE)  // rows at or past n_kept
@@ -401,10 +404,10 @@ __global__ void __launch_bounds__(kCoreThreads) second_pass_kernel(SecondArgs a)
       for (int h = 0; h < HP; ++h) {
         const int g = warp + 4 * h;
         if (g >= G) break;
-        const float p = expf(xt[h] + lwt - ls[h]);  // w / N_hat
+        const float p = expf(xt[h] + lwt - ls[h]);  // w / N_hat (RANGE: w)
         const float dist = dt[h];
         if constexpr (RANGE) {
-          if (tail) best[h] = fmaxf(best[h], sqrtf(omp) * p * sqrtf(dist));
+          if (tail) best[h] = fmaxf(best[h], sqrtf(omp) * (p / ln[h]) * sqrtf(dist));
         } else {
           if (row < n) a.out[(hq0 + g) * a.cap + row] = tail ? omp * p * p * dist : 0.f;
         }
@@ -483,8 +486,8 @@ static ebd_status launch_second(int head_dim, SecondArgs& a, int units, cudaStre
 }
 
 ebd_status launch_range_f32(int head_dim, const DecodeArgs& d, int units, cudaStream_t s) {
-  SecondArgs a = {d.Q, d.Kc, d.Vc, d.logw, d.n_kept, d.y, d.lse, d.b_t, d.cap, d.group,
-                  d.gstride, 1};
+  SecondArgs a = {d.Q, d.Kc, d.Vc, d.logw, d.n_kept, d.y, d.lse, d.radius, d.b_t, d.cap,
+                  d.group, d.gstride, 1};
   return launch_second<float, true>(head_dim, a, units, s);
 }
 
@@ -496,7 +499,7 @@ ebd_status launch_contributions_core(ebd_dtype dtype, int head_dim, int units, i
                                      const void* Q, const void* K_c, const void* V_c,
                                      const float* logw_c, const int32_t* n_kept, const float* y,
                                      const float* lse, float* contrib, cudaStream_t s) {
-  SecondArgs a = {Q, K_c, V_c, logw_c, n_kept, y, lse, contrib, cap, group, group, 1};
+  SecondArgs a = {Q, K_c, V_c, logw_c, n_kept, y, lse, nullptr, contrib, cap, group, group, 1};
   return dtype == EBD_F32 ? launch_second<float, false>(head_dim, a, units, s)
                           : launch_second<__nv_bfloat16, false>(head_dim, a, units, s);
 }

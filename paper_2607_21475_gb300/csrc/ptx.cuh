@@ -177,16 +177,6 @@ __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], uint32_t a0, uint3
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// D += A * B with the products' sum rounded to float32 before it is added (the
-// MMA starts from zero; accumulating in the tensor cores truncates).
-__device__ __forceinline__ void mma_add(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2,
-                                        uint32_t a3, uint32_t b0, uint32_t b1) {
-  float e[4] = {0.f, 0.f, 0.f, 0.f};
-  mma_bf16_16816(e, a0, a1, a2, a3, b0, b1);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) c[i] += e[i];
-}
-
 // Two floats -> packed bf16x2 (round to nearest even); `lo` goes to the low half.
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);

@@ -81,10 +81,16 @@ CASES = [
      (22.30e-7, 5.28e-7, 14.76e-7, 4.63e-7)),
     (32, 8, 4, 128, 1000, 1344, False, BF, 3.0, 2,
      (16.20e-7, 8.85e-7, 23.27e-7, 7.60e-7)),
+    (4, 8, 5, 128, 2460, 2953, True, BF, 3.0, 6,
+     (4.30e-7, 4.03e-7, 11.18e-7, 5.30e-7)),
+    (2, 8, 4, 128, 3000, 3333, True, BF, 3.0, 6,
+     (4.43e-7, 4.16e-7, 10.43e-7, 5.91e-7)),
     (4, 8, 2, 64, 9000, 9501, False, BF, 1.0, 6,
      (3.08e-7, 3.18e-7, 3.05e-7, 2.81e-7)),
     (4, 8, 8, 128, 1500, 1801, False, BF, 3.0, 6,
      (4.09e-7, 4.12e-7, 13.11e-7, 3.80e-7)),
+    (4, 8, 5, 128, 2460, 2960, True, BF, 3.0, 6,
+     (14.28e-7, 7.64e-7, 20.00e-7, 12.30e-7)),
 ]
 
 
