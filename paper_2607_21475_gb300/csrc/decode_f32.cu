@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(kCoreThreads) decode_f32_kernel(DecodeArgs a) 
           M[h] = mx;
         }
         if (lane == 0) fac[g] = f;
-        const float w = live ? expf(x - M[h]) : 0.f;
+        const float w = live ? expf((xs[g][lane] - M[h]) + lwt) : 0.f;
         const float u = omp * w * w, su = sq * w;
         l[h] += w;
         U[h] += u;
@@ -404,7 +404,7 @@ __global__ void __launch_bounds__(kCoreThreads) second_pass_kernel(SecondArgs a)
       for (int h = 0; h < HP; ++h) {
         const int g = warp + 4 * h;
         if (g >= G) break;
-        const float p = expf(xt[h] + lwt - ls[h]);  // w / N_hat (RANGE: w)
+        const float p = expf((xt[h] - ls[h]) + lwt);  // w / N_hat (RANGE: w)
         const float dist = dt[h];
         if constexpr (RANGE) {
           if (tail) best[h] = fmaxf(best[h], sqrtf(omp) * (p / ln[h]) * sqrtf(dist));

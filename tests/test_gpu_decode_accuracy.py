@@ -81,6 +81,10 @@ CASES = [
      (22.30e-7, 5.28e-7, 14.76e-7, 4.63e-7)),
     (32, 8, 4, 128, 1000, 1344, False, BF, 3.0, 2,
      (16.20e-7, 8.85e-7, 23.27e-7, 7.60e-7)),
+    (4, 8, 8, 128, 1000, 1100, False, F32, 3.0, 8,
+     (3.90e-7, 4.07e-7, 12.59e-7, 3.58e-7)),
+    (4, 8, 3, 64, 2000, 2200, True, F32, 3.0, 8,
+     (4.09e-7, 3.81e-7, 11.93e-7, 5.54e-7)),
     (4, 8, 5, 128, 2460, 2953, True, BF, 3.0, 6,
      (4.30e-7, 4.03e-7, 11.18e-7, 5.30e-7)),
     (2, 8, 4, 128, 3000, 3333, True, BF, 3.0, 6,
