@@ -224,23 +224,32 @@ __global__ void __launch_bounds__(kCtmWarps * 32)
     }
   }
   // per-head constants for the heads this lane's C fragments hold (2q, 2q + 1):
-  // ||y_hat - c||^2 and c . (y_hat - c), summed over the four lanes that hold a
-  // head's channels; and ||c||^2
+  // ||y_hat - c||^2 and c . (y_hat - c) with the y_hat - c that the MMA takes (hi +
+  // lo), so that the distance is the one to a y_hat of 16 bits and what these leave
+  // out meets v - y_hat only; summed over the four lanes that hold a head's
+  // channels; and ||c||^2.  Eight sums of D / 32 terms a lane, added as a tree
   float l2[2], yy[2], cy[2], cc = 0.f;
   {
-    float s2 = 0.f, sc = 0.f;
-    const float* yrow = y + (hq0 + (g < G ? g : 0)) * D;
+    float p2[8] = {}, pc[8] = {}, pq[8] = {};
 #pragma unroll
     for (int kk = 0; kk < D / 16; ++kk)
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const float c0 = -bf16_lo(cp[kk][h]), c1 = -bf16_hi(cp[kk][h]);
-        const float y0 = yrow[16 * kk + 8 * h + 2 * q] - c0;
-        const float y1 = yrow[16 * kk + 8 * h + 2 * q + 1] - c1;
-        s2 = fmaf(y0, y0, fmaf(y1, y1, s2));
-        sc = fmaf(c0, y0, fmaf(c1, y1, sc));
-        cc = fmaf(c0, c0, fmaf(c1, c1, cc));
-      }
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const int t = (4 * kk + 2 * h + i) & 7;
+          const float ce = -(i ? bf16_hi(cp[kk][h]) : bf16_lo(cp[kk][h]));
+          const float ye = i ? bf16_hi(yh[kk][h]) + bf16_hi(yl[kk][h])
+                             : bf16_lo(yh[kk][h]) + bf16_lo(yl[kk][h]);
+          p2[t] = fmaf(ye, ye, p2[t]);
+          pc[t] = fmaf(ce, ye, pc[t]);
+          pq[t] = fmaf(ce, ce, pq[t]);
+        }
+    const auto tree = [](const float (&x)[8]) {
+      return ((x[0] + x[1]) + (x[2] + x[3])) + ((x[4] + x[5]) + (x[6] + x[7]));
+    };
+    float s2 = tree(p2), sc = tree(pc);
+    cc = tree(pq);
 #pragma unroll
     for (int o = 1; o <= 2; o <<= 1) {
       s2 += __shfl_xor_sync(0xffffffffu, s2, o);

@@ -103,3 +103,38 @@ def test_errors_against_64_bits(E, B, H, G, d, rows, cap, exact, dtype, scale, s
     got = errors(E, B, H, G, d, rows, cap, exact, dtype, scale, seeds)
     for name, e, most in zip(("y", "lse", "V_hat", "b_t"), got, limits):
         assert e <= (1.10 if name == "V_hat" else 1.05) * most, (name, e, most)
+
+
+@pytest.mark.parametrize("B,H,G,d,rows,cap,mean,limit", [
+    (2, 8, 4, 128, 1500, 1808, 16.0, 8.76e-6),
+    (2, 8, 7, 128, 1500, 1808, 4.0, 3.24e-6),
+    (2, 8, 2, 64, 1500, 1808, 16.0, 13.12e-6),
+    (2, 8, 8, 128, 1500, 1808, 16.0, 18.96e-6),
+    (2, 8, 5, 128, 1500, 1808, 0.0, 1.57e-6),
+])
+def test_contributions_against_64_bits(E, B, H, G, d, rows, cap, mean, limit):
+    """The same for the contributions of given y_hat and log N_hat (2-norm over a
+    head), of values with a common mean; the limits are what head constants summed
+    over a whole warp left."""
+    errs = []
+    for seed in range(4):
+        g = torch.Generator(device=DEV).manual_seed(300 + seed)
+        rnd = lambda *s: torch.randn(s, generator=g, device=DEV)
+        K, V = rnd(B, H, cap, d).to(BF), (rnd(B, H, cap, d) + mean).to(BF)
+        lw = torch.rand((B, H, cap), generator=g, device=DEV) + 0.1
+        n = torch.full((B, H), rows, dtype=torch.int32, device=DEV)
+        Q = (2 * rnd(B, H * G, d)).to(BF)
+        ref = [reference(Q[b], K[b], V[b], lw[b], n[b], True) for b in range(B)]
+        y = torch.stack([r[0] for r in ref]).float()
+        lse = torch.stack([r[1] for r in ref]).float()
+        con = E.ebd_variance_contributions(Q, K, V, lw, n, y, lse)
+        for b in range(B):
+            q, k = Q[b].view(H, G, d).double(), K[b].double()
+            w = lw[b].double().unsqueeze(1)
+            p = torch.exp(q @ k.transpose(1, 2) / math.sqrt(d) + w - lse[b].view(H, G, 1).double())
+            dist = torch.stack([(V[b].double() - y[b].view(H, G, 1, d)[:, g_].double())
+                                .square().sum(-1) for g_ in range(G)], 1)
+            c = (-torch.expm1(-w) * p * p * dist)[..., :rows].flatten(0, 1)
+            e = (con[b, :, :rows].double() - c).norm(dim=-1) / c.norm(dim=-1)
+            errs.append(e)
+    assert float(torch.cat(errs).square().mean().sqrt()) <= limit
