@@ -108,6 +108,15 @@ __device__ __forceinline__ float one_minus_exp_neg(float x) {
   return 1.f - exp2f(-x * kLog2e);
 }
 
+// log2 x as the exponent and the log2 of a significand in [0.75, 1.5): the fast log2f
+// is within 2^-22 of its own result's size outside [0.5, 2], and low on average
+// (2.7e-7 at sums of some hundred).  0, infinities and NaN as log2f has them.
+__device__ __forceinline__ float log2_near_one(float x) {
+  if (!(x >= 1.17549435e-38f && x <= 3.40282347e+38f)) return log2f(x);
+  const int e = (__float_as_int(x) - 0x3f400000) >> 23;
+  return (float)e + log2f(__int_as_float(__float_as_int(x) - e * 0x800000));
+}
+
 __device__ __forceinline__ void raise_status(int32_t* st, int32_t bits) {
   if (st) atomicOr(st, bits);
 }

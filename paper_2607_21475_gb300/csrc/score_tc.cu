@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   }
   if (combines && rank == 0) {
     const int r = mt * kTcRows1 + row;
-    if (ok && r < a.n_obs) a.lse2[(size_t)unit * a.n_obs + r] = M * a.scale2 + log2f(tot);
+    if (ok && r < a.n_obs) a.lse2[(size_t)unit * a.n_obs + r] = M * a.scale2 + log2_near_one(tot);
   }
   if (!ok) raise_status(a.dev_status, EBD_DEV_TIMEOUT);
   tc_fence_before();

@@ -150,3 +150,25 @@ def test_a_unit_with_nan_leaves_its_neighbours_alone(E, R, N, d, dtype):
     E.ebd_score(q, K, got)
     assert torch.isfinite(ref).all()
     assert torch.equal(got[:, ::2], ref[:, ::2])
+
+
+@pytest.mark.parametrize("B,H,R,N,d,limit", [
+    (2, 4, 448, 5000, 64, 1.80e-7),     # keys over clusters of four
+    (1, 2, 800, 12001, 128, 3.02e-7),   # of eight, streamed query rows
+    (8, 4, 448, 6144, 128, 1.97e-7),    # one CTA per row tile
+])
+def test_scores_against_64_bits(E, B, H, R, N, d, limit):
+    """2-norm of the error over all scores; the limits are what one CTA per row tile
+    left on inputs drawn the same way (query rows beyond 512 on mma.sync)."""
+    errs = []
+    for seed in range(3):
+        g = torch.Generator(device=DEV).manual_seed(40 + seed)
+        K = torch.randn((B, H, N, d), generator=g, device=DEV).to(torch.bfloat16)
+        K[..., :4] *= 4
+        q = torch.randn((B, H, R, d), generator=g, device=DEV).to(torch.bfloat16)
+        s = E.ebd_score(q, K, torch.empty((B, H, N), device=DEV))
+        for b in range(B):
+            ref = torch.softmax(q[b].double() @ K[b].double().transpose(1, 2) / d ** 0.5, -1).sum(1)
+            errs.append((s[b].double() - ref).norm() / ref.norm())
+    e = float(torch.stack(errs).square().mean().sqrt())
+    assert e <= limit
