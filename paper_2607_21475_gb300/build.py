@@ -1,10 +1,11 @@
 """Build libebd.so (the C ABI of include/ebd.h) for GB300, in-tree.
 
 Each CUDA translation unit is compiled for sm_103a in parallel, then linked
-into ``paper_2607_21475_gb300/_build/libebd.so``; beside them the Python
-binding's native marshalling (``csrc/binding.cpp``, against the installed
-torch's headers) becomes ``_build/ebd_call.so``.  A content hash of the sources
-and flags skips the build when nothing changed.
+into ``paper_2607_21475_gb300/_build/libebd.so``, which needs the CUDA toolkit
+alone.  Where a torch with CUDA is installed, the Python binding's native
+marshalling (``csrc/binding.cpp``, against that torch's headers) becomes
+``_build/ebd_call.so`` beside it.  Content hashes of the sources and flags (for
+the latter also the versions of torch and Python) skip what has not changed.
 """
 from __future__ import annotations
 
@@ -40,30 +41,55 @@ def _sources():
     return sorted(os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".cu"))
 
 
-def _torch_version() -> str:
-    import torch
+def _torch():
+    """The installed torch, None without one or without CUDA in it."""
+    try:
+        import torch
+    except ImportError:
+        return None
+    return torch if torch.version.cuda else None
 
-    return torch.__version__
 
-
-def _digest(extra_flags) -> str:
+def _digest(files, extra) -> str:
     h = hashlib.sha256()
-    h.update(_torch_version().encode())
-    files = _sources() + sorted(os.path.join(CSRC, f) for f in os.listdir(CSRC)
-                                if f.endswith((".cuh", ".h", ".cpp")))
-    files.append(os.path.join(INCLUDE, "ebd.h"))
-    for f in files:
+    for f in [*files, os.path.join(INCLUDE, "ebd.h")]:
         h.update(f.encode())
         with open(f, "rb") as fh:
             h.update(fh.read())
-    h.update(" ".join(ARCH + NVCC_FLAGS + list(extra_flags)).encode())
+    h.update(" ".join(extra).encode())
     return h.hexdigest()
 
 
-def _build_call() -> None:
-    """The native marshalling of ebd.py, against this machine's torch and Python."""
-    import torch
+def _lib_digest(extra_flags) -> str:
+    return _digest(_sources() + sorted(os.path.join(CSRC, f) for f in os.listdir(CSRC)
+                                       if f.endswith((".cuh", ".h"))),
+                   ARCH + NVCC_FLAGS + list(extra_flags))
 
+
+def _call_digest(torch_version: str) -> str:
+    return _digest([os.path.join(CSRC, "binding.cpp")],
+                   [torch_version, sys.version, sysconfig.get_platform()])
+
+
+def _fresh(path: str, digest: str) -> bool:
+    """Whether `path` was built from what `digest` stands for."""
+    stamp = path[:-3] + ".stamp"
+    if not (os.path.exists(path) and os.path.exists(stamp)):
+        return False
+    with open(stamp) as fh:
+        return fh.read().strip() == digest
+
+
+def _stamp(path: str, digest: str) -> None:
+    with open(path[:-3] + ".stamp", "w") as fh:
+        fh.write(digest)
+
+
+def _build_call(torch, force: bool) -> None:
+    """The native marshalling of ebd.py, against this machine's torch and Python."""
+    dig = _call_digest(torch.__version__)
+    if not force and _fresh(CALL, dig):
+        return
     cuda = os.path.dirname(os.path.dirname(_nvcc()))
     tdir = os.path.dirname(torch.__file__)
     tinc, tlib = os.path.join(tdir, "include"), os.path.join(tdir, "lib")
@@ -78,17 +104,19 @@ def _build_call() -> None:
     if r.returncode != 0:
         raise RuntimeError(f"g++ failed for binding.cpp:\n{r.stderr}")
     os.replace(tmp, CALL)
+    _stamp(CALL, dig)
 
 
 def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
-    """Compile the CUDA sources and link libebd.so; returns the library path."""
+    """Compile the CUDA sources and link libebd.so (and, with a torch to build it
+    against, the binding); returns the library path."""
     os.makedirs(BUILD, exist_ok=True)
-    stamp = os.path.join(BUILD, "libebd.stamp")
-    dig = _digest(extra_flags)
-    if not force and os.path.exists(LIB) and os.path.exists(CALL) and os.path.exists(stamp):
-        with open(stamp) as fh:
-            if fh.read().strip() == dig:
-                return LIB
+    torch = _torch()
+    dig = _lib_digest(extra_flags)
+    if not force and _fresh(LIB, dig):
+        if torch is not None:
+            _build_call(torch, force)
+        return LIB
     nvcc = _nvcc()
     srcs = _sources()
     objs = [os.path.join(BUILD, os.path.basename(s)[:-3] + ".o") for s in srcs]
@@ -104,17 +132,17 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
         return obj
 
     with ThreadPoolExecutor(max_workers=min(len(srcs) + 1, os.cpu_count() or 4)) as ex:
-        call = ex.submit(_build_call)
+        call = ex.submit(_build_call, torch, force) if torch is not None else None
         list(ex.map(compile_one, zip(srcs, objs)))
-        call.result()
+        if call is not None:
+            call.result()
     tmp = LIB + ".tmp"
     cmd = [nvcc, *ARCH, "-shared", "-cudart", "static", "-o", tmp, *objs]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"link of libebd.so failed:\n{r.stderr}")
     os.replace(tmp, LIB)
-    with open(stamp, "w") as fh:
-        fh.write(dig)
+    _stamp(LIB, dig)
     return LIB
 
 

@@ -8,7 +8,8 @@ contiguity, passes raw pointers plus sizes, and raises ``EbdError`` on a
 non-OK status.  Every step of the hot path runs in the library's CUDA
 kernels.  PyTorch supplies device memory and the current stream.
 
-The calls of a decode loop go through ``ebd_call`` (csrc/binding.cpp), which
+The calls of a decode loop go through ``ebd_call`` (csrc/binding.cpp, built
+wherever torch has CUDA), which
 does the same checks and the call natively on plain dense CUDA tensors and the
 current stream; whatever it does not take (it then calls nothing) goes through
 the Python checks below, which handle the call or raise.
@@ -156,11 +157,22 @@ def lib():
     return _LIB
 
 
+class _PythonOnly:
+    """Stands for ebd_call where it was not built (a torch without CUDA): takes no
+    call, so that every one goes the Python way."""
+
+    def __getattr__(self, name):
+        return lambda *args: None
+
+
 def _call():
     """The native marshalling module, loaded and bound to the library once."""
     global _CALL
     if _CALL is None:
         L = lib()
+        if not os.path.exists(CALL):
+            _CALL = _PythonOnly()
+            return _CALL
         loader = importlib.machinery.ExtensionFileLoader("ebd_call", CALL)
         mod = importlib.util.module_from_spec(importlib.util.spec_from_loader("ebd_call", loader))
         loader.exec_module(mod)
