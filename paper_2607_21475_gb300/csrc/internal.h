@@ -5,9 +5,14 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/ebd.h"
 
 namespace ebd {
+
+// Number of SMs of the current device (cached per device).
+int sm_count();
 
 inline ebd_status cuda_status(cudaError_t e) { return e == cudaSuccess ? EBD_OK : EBD_ERR_CUDA; }
 
@@ -21,6 +26,37 @@ template <typename Kernel>
 ebd_status allow_smem(Kernel kernel, int most) {
   return cuda_status(
       cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+}
+
+// Clusters of 2^lg CTAs (lg < 4) of Kernel that the current device holds at a time.  A
+// cluster lies within one GPC, so for the larger ones that is fewer than SMs / 2^lg
+// (152 SMs hold 15 clusters of 8 whose CTAs take an SM each).  Asked once per
+// device and kernel; `smem`: dynamic shared memory of a CTA, `most`: allow_smem's.
+template <auto Kernel>
+int resident_clusters(int lg, int threads, int smem, int most) {
+  static std::atomic<int> cached[64][4];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return sm_count() >> lg;
+  int n = cached[dev][lg].load(std::memory_order_relaxed);
+  if (n > 0) return n;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(1u << lg);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 1u << lg;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (allow_smem(Kernel, most) != EBD_OK ||
+      cudaOccupancyMaxActiveClusters(&n, Kernel, &cfg) != cudaSuccess || n < 1) {
+    (void)cudaGetLastError();
+    n = sm_count() >> lg;
+  }
+  cached[dev][lg].store(n, std::memory_order_relaxed);
+  return n;
 }
 
 // Launch as a programmatic dependent of what precedes it in the stream (the
@@ -42,9 +78,6 @@ ebd_status launch_dependent(void (*kernel)(Params...), dim3 grid, int threads, s
 }
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
-
-// Number of SMs of the current device (cached per device).
-int sm_count();
 
 // Design validation shared by the eviction entry points (evict.cu).
 ebd_status check_design(const ebd_design* d);

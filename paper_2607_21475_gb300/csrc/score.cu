@@ -14,8 +14,6 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
-#include <atomic>
-
 #include "common.cuh"
 #include "internal.h"
 #include "ptx.cuh"
@@ -369,39 +367,6 @@ static ebd_status launch_f32(Kernel kernel, long long grid, int cluster, int sme
   return cuda_status(cudaLaunchKernelEx(&cfg, kernel, args...));
 }
 
-// Clusters of 2^lg CTAs of pass 1 that this GPU holds at a time (a cluster lies
-// within one GPC, so that is fewer than SMs / 2^lg; at d = 64 two CTAs share an
-// SM), asked once per device and kernel.
-template <int D, int I>
-static int resident_lse_clusters(int lg) {
-  static std::atomic<int> cached[64][4];
-  const auto kernel = score_lse_f32_kernel<D, I>;
-  const int cluster = 1 << lg, smem = F32Layout<D, I>::kLseBytes;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return sm_count() >> lg;
-  int n = cached[dev][lg].load(std::memory_order_relaxed);
-  if (n > 0) return n;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)cluster);
-  cfg.blockDim = dim3(kFThreads);
-  cfg.dynamicSmemBytes = smem;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)cluster;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
-          cudaSuccess ||
-      cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n < 1) {
-    (void)cudaGetLastError();
-    n = sm_count() >> lg;
-  }
-  cached[dev][lg].store(n, std::memory_order_relaxed);
-  return n;
-}
-
 // Pass 1 with 8 I rows per tile: its cost in microseconds (waves x (start-up +
 // key tiles at `tile_us`)) with the best split of the keys over C CTAs.
 template <int D, int I>
@@ -412,7 +377,9 @@ static double plan_lse_f32(int units, int n_ctx, int n_obs, double tile_us, int&
   for (int lg = 0; lg < 4; ++lg) {
     const int c = 1 << lg;
     if (lg > 0 && c > ktiles) break;
-    const long long fit = resident_lse_clusters<D, I>(lg);
+    // (at d = 64 two CTAs share an SM)
+    constexpr int kSmem = F32Layout<D, I>::kLseBytes;
+    const long long fit = resident_clusters<score_lse_f32_kernel<D, I>>(lg, kFThreads, kSmem, kSmem);
     const double cost = (double)((rts + fit - 1) / fit) * (3. + tile_us * ((ktiles + c - 1) / c));
     if (lg == 0 || cost < best) {
       best = cost;

@@ -963,10 +963,14 @@ static ebd_status launch_score_tc_t(int units, int n_ctx, int n_obs, const void*
   // start-up: the query tile, the first key tile and the cluster's combine).
   // 8 units x 1024 rows x 8189 keys on 128 instead of 64 CTAs: 18.7 us
   const int nk = (n_ctx + kTcKeys1 - 1) / kTcKeys1;
-  int C = 1;
-  while (C < 8 && (long long)units * a.mtiles * 2 * C <= sm_count() && nk >= 8 * C) C *= 2;
-  a.csize = C;
   const int smem1 = Tc1Layout<D>::kBytes;
+  int C = 1;
+  for (int lg = 1; lg < 4 && nk >= 4 << lg &&
+                   (long long)units * a.mtiles <=
+                       resident_clusters<score_lse_tc_kernel<D>>(lg, kTcThreads, smem1, smem1);
+       ++lg)
+    C = 1 << lg;
+  a.csize = C;
   ebd_status st = launch_tc_kernel(score_lse_tc_kernel<D>, units * a.mtiles * C, kTcThreads, C,
                                    smem1, s, tmQ1, tmK1, a);
   if (st != EBD_OK && C > 1) {  // the cluster could not be placed: one CTA per row tile

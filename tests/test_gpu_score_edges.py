@@ -172,3 +172,29 @@ def test_scores_against_64_bits(E, B, H, R, N, d, limit):
             errs.append((s[b].double() - ref).norm() / ref.norm())
     e = float(torch.stack(errs).square().mean().sqrt())
     assert e <= limit
+
+
+@pytest.mark.parametrize("few,many", [(16, 20), (38, 40)])
+def test_fewer_row_tiles_take_no_longer(E, few, many):
+    """Row tiles whose keys are split over clusters of a size that the device does
+    not hold for all of them at once would wait for a second wave: 16 of them
+    then take longer than 20, whose clusters are half the size."""
+    def microseconds(units, N=8192, d=128, R=128):
+        g = torch.Generator(device=DEV).manual_seed(1)
+        K = torch.randn((units, 1, N, d), generator=g, device=DEV).to(torch.bfloat16)
+        q = torch.randn((units, 1, R, d), generator=g, device=DEV).to(torch.bfloat16)
+        s = torch.empty((units, 1, N), device=DEV)
+        ws = torch.empty(E.ebd_score_workspace_bytes(units, 1, R), dtype=torch.uint8, device=DEV)
+        best = float("inf")
+        for _ in range(7):
+            t0, t1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            for k in range(60):
+                if k == 10:
+                    t0.record()
+                E.ebd_score(q, K, s, ws)
+            t1.record()
+            torch.cuda.synchronize()
+            best = min(best, t0.elapsed_time(t1) * 20)
+        return best
+
+    assert microseconds(few) <= 1.03 * microseconds(many)
