@@ -2,7 +2,7 @@
 //     s_j = sum_r softmax_j(q_r . K^T / sqrt(d))
 // (Appendix B harness, H2O-style accumulated attention from R observation
 // query rows of a KV head's group), bf16 inputs, f32 accumulation in tensor
-// memory, head_dim 64/128, any R.
+// memory, head_dim 64/128, R up to 4096.
 //
 // Pass 1, score_lse_tc_kernel: one CTA per (unit, 128 query rows), or a
 // cluster of 2-8 CTAs that split the unit's keys where that leaves SMs idle
@@ -800,7 +800,8 @@ __global__ void __launch_bounds__(kTsThreads, 1)
           break;
         }
         tc_fence_after();
-        // this quarter's 16, 32, 48 or 64 columns of the chunk
+        // this quarter's 48 or 64 columns of the chunk: nine blocks or more in
+        // ceil(blocks / 4) chunks are three or four each
         const int pc = block0(c), nb = block0(c + 1) - pc;
         const uint32_t tbase = tlane + b * kTsCols + party * 16 * nb;
         const float4* l4 = reinterpret_cast<const float4*>(lse_s + pc * 64 + party * 16 * nb);
@@ -812,9 +813,7 @@ __global__ void __launch_bounds__(kTsThreads, 1)
           sum += exp_sum(r, a.scale2, [&](int q) { return l4[q]; });
         };
         if (nb == 4) take(std::integral_constant<int, 64>{});
-        else if (nb == 3) take(std::integral_constant<int, 48>{});
-        else if (nb == 2) take(std::integral_constant<int, 32>{});
-        else take(std::integral_constant<int, 16>{});
+        else take(std::integral_constant<int, 48>{});
       }
       if (!ok) break;
       // the first quarter's warps add the four parts, in order

@@ -1,7 +1,9 @@
-"""Accumulated-attention scores at the edges of the tensor-core kernels' tiles
-(160-key tiles, 128-key items, chunks of at most 160 query rows, query rows
-resident up to 512 and streamed beyond, keys split over a cluster) and of the
-float32 kernels' tiles, against the float64 oracle."""
+"""Accumulated-attention scores at the edges of the tensor-core kernels' tiles (pass
+1: 128 query rows x 256 keys, the key tiles split over a cluster of up to eight
+CTAs with at least four each; pass 2: 128 keys, up to 512 query rows in two
+accumulators of 256 columns and 32-column steps, beyond that 64-row blocks in
+chunks of three or four) and of the float32 kernels' (32 or 64 rows x 128 keys),
+against the float64 oracle."""
 import os
 import subprocess
 import sys
@@ -41,17 +43,27 @@ def check(E, B, H, R, N, d, dtype, units=None):
 
 
 @pytest.mark.parametrize("B,H,R,N,d", [
-    (1, 1, 160, 160, 128),     # one full chunk, one full key tile
-    (1, 2, 161, 161, 128),     # one row and one key past them
-    (2, 1, 320, 159, 64),      # two chunks: two of the three groups take part
-    (1, 2, 480, 481, 128),     # three chunks, four key tiles
-    (1, 2, 513, 127, 128),     # the fewest streamed rows; under one item of keys
-    (1, 1, 1024, 641, 64),     # seven chunks, five key tiles and a key
+    (1, 1, 128, 256, 128),     # one full row tile and key tile, two items
+    (1, 2, 129, 257, 128),     # one row and one key past them
+    (2, 1, 256, 255, 64),      # a full accumulator; a key short of a tile
+    (1, 2, 257, 128, 128),     # a row in the second accumulator; one item
+    (1, 1, 512, 129, 64),      # two full accumulators; a key in a second item
+    (1, 1, 160, 160, 128),     # five steps of columns; part of a second item
+    (1, 2, 161, 161, 128),
+    (2, 1, 320, 159, 64),      # a second accumulator of 64 columns
+    (1, 2, 480, 481, 128),     # of 224; four items
+    (1, 2, 513, 127, 128),     # the fewest streamed rows: three chunks of three blocks
+    (1, 1, 640, 257, 64),      # three, three and four
+    (1, 1, 1024, 641, 64),     # four chunks of four; five items and a key
+    (1, 2, 1025, 256, 128),    # a row in a seventeenth block: 3, 3, 4, 3, 4
     (1, 1, 4096, 129, 128),    # the most rows
     (40, 8, 33, 130, 128),     # more units than CTAs: several units and items per CTA
     (24, 8, 520, 40, 64),      # the same with streamed rows
-    (1, 1, 100, 2561, 128),    # keys over a cluster of two CTAs, the last tile one key
-    (1, 2, 449, 10241, 64),    # over a cluster of eight
+    (1, 1, 100, 1793, 128),    # eight key tiles, the last of one key: a cluster of two
+    (1, 1, 100, 1792, 128),    # seven: no split
+    (1, 1, 100, 2561, 128),
+    (1, 2, 449, 10241, 64),    # a cluster of eight
+    (2, 8, 100, 8192, 64),     # 16 row tiles: more than there are clusters of eight
 ])
 def test_tensor_core_scores_at_tile_edges(E, B, H, R, N, d):
     units = None if B * H < 16 else (0, 1, B * H // 2, B * H - 1)
@@ -62,8 +74,8 @@ def test_tensor_core_scores_at_tile_edges(E, B, H, R, N, d):
     (1, 1, 64, 128, 128),      # one full row tile, one full key tile
     (1, 2, 65, 129, 64),       # one row and one key past them
     (1, 1, 1, 1, 64),
-    (2, 3, 130, 1023, 128),    # keys over a cluster of four CTAs
-    (1, 1, 63, 4097, 128),     # over a cluster of eight, the last tile one key
+    (2, 3, 130, 1023, 128),    # keys over a cluster, the last tile a key short
+    (1, 1, 63, 4097, 128),     # the last tile one key
     (40, 8, 70, 130, 64),      # more row tiles than SMs
 ])
 def test_float32_scores_at_tile_edges(E, B, H, R, N, d):
